@@ -405,7 +405,9 @@ __global__ void sum_parts_kernel(const double *part, int slices, int n_models, d
 // order and compared, so the decision always equals the all-FP64 one.
 
 // FP64 objective of node u's label s, summed in neighbour order; the loads of
-// kSumBatch neighbours at a time are independent of each other.
+// kSumBatch neighbours at a time are independent of each other.  A neighbour that
+// a team no longer waits for (ERR_TIMEOUT is set) may still be undecided, -1: it
+// counts as label 0 here too.
 constexpr int kSumBatch = 8;
 __device__ double round_sum64(const InRec *rec, int K, const int *labels, const float *tab, const ulonglong2 *msg,
                               double a, int s)
@@ -416,7 +418,7 @@ __device__ double round_sum64(const InRec *rec, int K, const int *labels, const 
         for (int j = 0; j < kSumBatch; ++j)
             if (k0 + j < K) {
                 const InRec r = rec[k0 + j];
-                const int xv = *reinterpret_cast<const volatile int *>(labels + r.gu);
+                const int xv = max(*reinterpret_cast<const volatile int *>(labels + r.gu), 0);
                 t[j] = (static_cast<double>(tab[r.toff + static_cast<long long>(xv) * r.ld + s]) - se_d(msg[r.mu + xv])) -
                        se_d(msg[r.mv + s]);
             }
