@@ -737,8 +737,10 @@ static mplpp_status apply_mapping(mplpp_solver *s, int C, int T, int want)
             apply_resident_mapping(s, 0, optin) == MPLPP_OK)
             return MPLPP_OK;
         if (want != MPLPP_MODE_LOOPED && apply_narrow_mapping(s) == MPLPP_OK) return MPLPP_OK;
-        s->err.clear();
+        if (T != 32) s->err.clear();
     }
+    // (a CTA of the cluster drivers splits its warps between the two node vectors)
+    if (T == 32) return s->err.empty() ? fail(s, MPLPP_E_UNSUPPORTED, "32 threads: the narrow form only") : MPLPP_E_UNSUPPORTED;
     mapping_for(s, C, T);
     int C1 = 0, T1 = 0;  // the persistent driver's own choice for narrow rows
     if (want != MPLPP_MODE_LOOPED && T == 0 && s->opt.cluster == 0 && s->opt.threads == 0 && narrow_rows(s, &C1, &T1)) {
