@@ -276,8 +276,12 @@ typedef struct {
     int64_t edges;              /* total edges over all models                                */
     int32_t phases;             /* matchings per iteration (max over models)                 */
     int32_t mode;               /* MPLPP_MODE_LOOPED or _PERSISTENT actually used             */
-    int32_t cluster;            /* CTAs per edge                                              */
-    int32_t threads;            /* threads per CTA                                            */
+    int32_t cluster;            /* CTAs per edge; 0: the persistent driver's narrow form (up to 32
+                                   labels), a group of lanes per edge                         */
+    int32_t threads;            /* threads per CTA; 0: one warp per CTA where options.threads
+                                   cannot ask for that (the narrow form, the resident driver on
+                                   small models).  A solver created with these mode, cluster and
+                                   threads takes the same mapping                             */
     int32_t grid;               /* persistent mode: CTAs launched                             */
     int32_t launches_per_iteration; /* kernel launches one iteration takes (looped: phases)   */
     int32_t labeling_launches;  /* kernel launches of one mplpp_labeling: the rounding, the

@@ -1494,6 +1494,12 @@ static const char *mode_name(int mode)
                                            : "looped";
 }
 
+// A mapping as options.cluster and options.threads name it, so that what info and
+// the autotuner report can be asked for.  The narrow form and a resident block of
+// one warp (32 threads) have no name there: they are what 0 chooses.
+static int option_cluster(int mode, int C, int T) { return mode == MPLPP_MODE_PERSISTENT && T == 32 ? 0 : C; }
+static int option_threads(int mode, int T) { return T == 32 && mode != MPLPP_MODE_WARP ? 0 : T; }
+
 // Measured choice of the mapping: every feasible (CTAs per edge, threads per
 // CTA, driver) runs `iterations` iterations of the solver's own models from
 // the same state, timed with CUDA events on the solver's stream; the fastest
@@ -1603,12 +1609,14 @@ extern "C" mplpp_status mplpp_autotune(mplpp_solver *s, int32_t iterations, char
     CK(s, cudaStreamSynchronize(st));
     if (report && report_size) {
         std::string r = "{\"iterations\": " + std::to_string(iterations) + ", \"best\": {\"cluster\": " +
-                        std::to_string(best.C) + ", \"threads\": " + std::to_string(best.T) + ", \"mode\": \"" +
+                        std::to_string(option_cluster(best.mode, best.C, best.T)) + ", \"threads\": " +
+                        std::to_string(option_threads(best.mode, best.T)) + ", \"mode\": \"" +
                         mode_name(best.mode) + "\", \"ms\": " +
                         std::to_string(best.ms) + "}, \"candidates\": [";
         for (size_t i = 0; i < done.size(); ++i)
-            r += std::string(i ? ", " : "") + "[" + std::to_string(done[i].C) + ", " + std::to_string(done[i].T) +
-                 ", \"" + mode_name(done[i].mode) + "\", " +
+            r += std::string(i ? ", " : "") + "[" +
+                 std::to_string(option_cluster(done[i].mode, done[i].C, done[i].T)) + ", " +
+                 std::to_string(option_threads(done[i].mode, done[i].T)) + ", \"" + mode_name(done[i].mode) + "\", " +
                  std::to_string(done[i].ms) + "]";
         r += "]}";
         std::snprintf(report, report_size, "%s", r.c_str());
@@ -1624,8 +1632,8 @@ extern "C" mplpp_status mplpp_info(const mplpp_solver *s, mplpp_info_t *info)
     info->edges = s->EE;
     info->phases = s->P;
     info->mode = s->struct_auto ? MPLPP_MODE_STRUCTURED : s->mode;
-    info->cluster = s->C;
-    info->threads = s->T;
+    info->cluster = option_cluster(s->mode, s->C, s->T);
+    info->threads = option_threads(s->mode, s->T);
     info->grid = s->mode == MPLPP_MODE_PERSISTENT ? s->clusters * s->C
                  : s->mode == MPLPP_MODE_WARP     ? s->warp_blocks
                  : (s->mode == MPLPP_MODE_QUEUE || s->mode == MPLPP_MODE_STRUCTURED_QUEUE) ? s->queue_blocks
