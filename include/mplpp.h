@@ -45,7 +45,7 @@ typedef enum {
     MPLPP_E_INVALID = -1,     /* bad argument: sizes, edge order, duplicate edge, bad schedule */
     MPLPP_E_NOMEM = -2,       /* host or device allocation failed                              */
     MPLPP_E_CUDA = -3,        /* a CUDA runtime call failed (message has the CUDA error)       */
-    MPLPP_E_TIMEOUT = -4,     /* a device-side wait exceeded options.spin_limit polls          */
+    MPLPP_E_TIMEOUT = -4,     /* a device-side wait ran out (options.spin_limit)               */
     MPLPP_E_NONFINITE = -5,   /* a result is NaN or infinite                                   */
     MPLPP_E_STATE = -6,       /* call not valid in the current state (e.g. backward w/o record) */
     MPLPP_E_UNSUPPORTED = -7  /* a shape beyond a compiled limit, or a driver / update / cost
@@ -160,7 +160,8 @@ typedef struct {
                                  than will ever happen, so the bounded wait must run out and the
                                  run must end with MPLPP_E_TIMEOUT instead of hanging            */
     int32_t rule;             /* MPLPP_RULE_* (0 = the Handshake update)                        */
-    int64_t spin_limit;       /* polls before a device-side wait gives up with MPLPP_E_TIMEOUT */
+    int64_t spin_limit;       /* polls before a device-side wait gives up with MPLPP_E_TIMEOUT;
+                                 at least 2^22 for the structured driver that AUTO takes       */
     int32_t test_backward;    /* testing only (0 otherwise), bit flags for mplpp_backward:
                                  1 = replay every minimization in FP64 instead of screening
                                  it in FP32 first; 2 = checkpoints and a second replay per
@@ -170,7 +171,7 @@ typedef struct {
 } mplpp_options;
 
 /* Fills *opt with defaults: AUTO mode, graphs on, host inputs, no record,
- * automatic mapping, spin_limit = 2^26 (well above any legitimate wait). */
+ * automatic mapping, spin_limit = 2^22 (well above any legitimate wait). */
 void mplpp_options_default(mplpp_options *opt);
 
 /* Builds an edge schedule (Sec. 6, Alg. 1) for one graph.

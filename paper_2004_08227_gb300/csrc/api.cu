@@ -1169,7 +1169,7 @@ cudaError_t enqueue_persistent(mplpp_solver *s, cudaStream_t st, int iterations)
         sp.iterations = iterations;
         sp.test_wait = s->opt.test_unreachable_wait ? 1 : 0;
         sp.err = s->d_err;
-        sp.spin_limit = s->opt.spin_limit;
+        sp.spin_limit = s->struct_auto ? s->own_wait_limit() : s->opt.spin_limit;
         return launch_struct_queue(sp, s->queue_blocks, st);
     }
     if (s->mode == MPLPP_MODE_RESIDENT) {  // reads values only, writes version 0: no restamp

@@ -1,5 +1,6 @@
 // solver.h -- the opaque mplpp_solver (host bookkeeping + device buffers).
 #pragma once
+#include <algorithm>
 #include <cstdint>
 #include <memory>
 #include <string>
@@ -35,6 +36,14 @@ struct mplpp_solver {
     cudaStream_t cap_stream = nullptr;
     bool stream_ok = false;
     mplpp_options opt = {};
+    // Polls of the waits that no caller asked for (the automatic structured driver,
+    // the rounding, the backward): options.spin_limit, but not below 2^22 (seconds),
+    // so that a low limit set for a driver's waits does not end these.  Tests of
+    // waits that run out take the limit as it is.
+    long long own_wait_limit() const
+    {
+        return opt.test_unreachable_wait ? opt.spin_limit : std::max<long long>(opt.spin_limit, 1LL << 22);
+    }
     std::string err;
     std::vector<mplpp::ModelHost> models;
 

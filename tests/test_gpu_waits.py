@@ -37,3 +37,16 @@ def test_rounding_after_a_timed_out_run_without_sync(n, labels):
             good.run(2)
             x, _ = good.labeling()
             assert (x >= 0).all() and (x < m.labels).all()
+
+
+def test_a_low_limit_leaves_the_automatic_structured_driver_alone():
+    """spin_limit = 1 ends waits of the drivers that a caller asked for; AUTO's
+    structured driver took a launch per matching, without waits, before it ran
+    from the queue."""
+    m = W.grid_trunc_linear(12, 13, 20, weight=1.0, tau=4.0, seed=1)
+    with Solver([m], spin_limit=1) as a, Solver([m], mode="looped") as b:
+        assert a.info()["mode"] == "structured" and a.info()["launches_per_iteration"] == 0
+        a.run(20)
+        b.run(20)
+        a.sync()
+        assert all(np.array_equal(x, y) for x, y in zip(a.state_arrays()[1:], b.state_arrays()[1:]))
