@@ -155,13 +155,16 @@ typedef struct {
     int32_t cluster;          /* CTAs sharing one edge (1..8); 0 = chosen from the shapes      */
     int32_t threads;          /* threads per CTA: 0 = chosen from the shapes, else a multiple
                                  of 32 in 64..512 (32..512 for MPLPP_MODE_WARP)                */
-    int32_t test_unreachable_wait; /* testing only (0 otherwise): in the persistent driver the
+    int32_t test_unreachable_wait; /* testing only (0 otherwise): in the persistent drivers the
                                  first edge of the first worker waits for one node update more
-                                 than will ever happen, so the bounded wait must run out and the
-                                 run must end with MPLPP_E_TIMEOUT instead of hanging            */
+                                 than will ever happen, as does the backward's first update, and
+                                 the rounding's last node for labels that it never sees; the
+                                 bounded wait must run out after spin_limit polls and the call
+                                 end with MPLPP_E_TIMEOUT instead of hanging                     */
     int32_t rule;             /* MPLPP_RULE_* (0 = the Handshake update)                        */
     int64_t spin_limit;       /* polls before a device-side wait gives up with MPLPP_E_TIMEOUT;
-                                 at least 2^22 for the structured driver that AUTO takes       */
+                                 at least 2^22 for the structured driver that AUTO takes, the
+                                 rounding and the backward                                    */
     int32_t test_backward;    /* testing only (0 otherwise), bit flags for mplpp_backward:
                                  1 = replay every minimization in FP64 instead of screening
                                  it in FP32 first; 2 = checkpoints and a second replay per

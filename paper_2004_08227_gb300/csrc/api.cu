@@ -1303,7 +1303,8 @@ extern "C" mplpp_status mplpp_labeling(mplpp_solver *s, int32_t *labels, double 
     s->err.clear();
     CK(s, launch_round(s->d_edges, s->d_nodes, s->N, s->d_in_off, s->d_in_rec, s->d_round_order, s->d_mnode_off,
                        s->d_medge_off, static_cast<int>(s->models.size()), s->d_tab, s->d_agg, s->d_msg, s->d_un0,
-                       s->d_labels, s->d_energy, s->d_err, s->max_label, s->max_terms, s->d_part, s->stream));
+                       s->d_labels, s->d_energy, s->d_err, s->max_label, s->max_terms, s->d_part, s->own_wait_limit(),
+                       s->opt.test_unreachable_wait, s->stream));
     CK(s, cudaMemcpyAsync(labels, s->d_labels, sizeof(int) * s->N, cudaMemcpyDeviceToHost, s->stream));
     if (energy)
         CK(s, cudaMemcpyAsync(energy, s->d_energy, sizeof(double) * s->models.size(), cudaMemcpyDeviceToHost,

@@ -281,7 +281,8 @@ __global__ void __launch_bounds__(kThreads) bw_sweep_kernel(BwQueue p, const uns
             const int j = tid + c * T;
             cb[c] = uhb[c] = bb[c] = vhb[c] = 0.0;
             if (j < Lu) {
-                const double Pu = bw_poll_diff(p, p.agg + ed.au + j, p.msg + ed.mu + j, vu, ve, drain, &uhb[c]);
+                const double Pu = bw_poll_diff(p, p.agg + ed.au + j, p.msg + ed.mu + j, g > 0 ? vu : vu + p.test_wait, ve,
+                                               drain, &uhb[c]);
                 cb[c] = uhb[c] + Pu;
             }
             if (j < Lv) {
@@ -620,7 +621,8 @@ extern "C" mplpp_status mplpp_backward(mplpp_solver *s, const float *dD, float *
     q.rec_stride = s->rec_stride;
     q.queue = s->d_bw_queue;
     q.err = s->d_err;
-    q.spin_limit = std::max<long long>(s->opt.spin_limit, 1LL << 22);
+    q.spin_limit = s->own_wait_limit();
+    q.test_wait = s->opt.test_unreachable_wait ? 1u : 0u;
     q.lmax = lmax;
     // `n` iterations of the FP64 replay, `done` of them already in the state; rec:
     // the records of the first one, or nullptr

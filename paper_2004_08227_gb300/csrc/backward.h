@@ -44,6 +44,7 @@ struct BwQueue {
     int *err;
     long long spin_limit;
     int lmax;
+    unsigned test_wait;      // testing: 1 if the first update waits for one of node u that never comes
 };
 #ifdef __CUDACC__
 // Place g of the queue: iteration and item (in 32 bits: launches hold fewer than

@@ -451,7 +451,7 @@ __device__ __forceinline__ void warp_low_label(double &best, int &bi)
 // trip for the label, one for its table row and the argmin, instead of a walk
 // over all of a node's neighbours or a launch per level.  A team waits only
 // for nodes taken earlier by running teams, so the waits end; they are bounded
-// all the same (kRoundSpin polls, then ERR_TIMEOUT and no more waiting).
+// all the same (spin_limit polls, then ERR_TIMEOUT and no more waiting).
 // A team is one warp for nodes of at most 32 NL labels, else TW warps of 32 NL
 // labels each (TW > 1: the whole block).  With at most 16 labels the lanes split
 // into 32 / G groups of G, each adding its share of the neighbours.
@@ -465,7 +465,6 @@ __device__ __forceinline__ void warp_low_label(double &best, int &bi)
 // 1.15 -> 1.04 ms, the grid 0.63 -> 0.57 ms, kNN 191 -> 170 us, 16 K_50 with 64
 // labels 89 -> 82 us (8 or 16 neighbours: K_600 1.06, 1.11 ms; with wider labels,
 // a block per node, nothing: 85 us).
-constexpr int kRoundSpin = 1 << 22;
 constexpr int kRoundFetch = 4;  // the last undecided neighbours, fetched ahead
 constexpr int kRoundWarps = 4;  // warps per block of one-warp teams
 constexpr int kRoundMaxWarps = 16;
@@ -473,7 +472,8 @@ constexpr int kRoundMaxWarps = 16;
 template <int NL, bool TEAM>
 __global__ void __launch_bounds__(TEAM ? 32 * kRoundMaxWarps : 32 * kRoundWarps)
     round_flow_kernel(const NodeDesc *nodes, const int *order, int n_nodes, const int *in_off, const InRec *in_rec,
-                      const float *tab, const ulonglong2 *agg, const ulonglong2 *msg, int *labels, int *queue, int *err)
+                      const float *tab, const ulonglong2 *agg, const ulonglong2 *msg, int *labels, int *queue, int *err,
+                      long long spin_limit, int test_wait)
 {
     constexpr unsigned kAll = 0xffffffffu;
     constexpr int kRows = NL == 1 ? 8 : (NL == 2 ? 4 : 2);  // neighbours whose loads are in flight together
@@ -521,11 +521,12 @@ __global__ void __launch_bounds__(TEAM ? 32 * kRoundMaxWarps : 32 * kRoundWarps)
             InRec r = {};
             if (on) r = rec[b + lane];
             unsigned pending = __ballot_sync(kAll, on);
-            int spins = 0;
+            long long spins = 0;
             bool fetched = false;
             while (pending) {
                 int x = -1;
                 if ((pending >> lane) & 1u) x = *reinterpret_cast<volatile int *>(labels + r.gu);
+                if (test_wait && ticket == n_nodes - 1) x = -1;  // testing: the last node sees no label
                 if (drain && x < 0) x = 0;
                 unsigned ready = __ballot_sync(kAll, x >= 0) & pending;
                 if (!ready) {
@@ -543,7 +544,7 @@ __global__ void __launch_bounds__(TEAM ? 32 * kRoundMaxWarps : 32 * kRoundWarps)
                         }
                         continue;
                     }
-                    if (++spins > kRoundSpin || ((spins & 255) == 0 && *reinterpret_cast<volatile int *>(err) == ERR_TIMEOUT)) {
+                    if (++spins > spin_limit || ((spins & 255) == 0 && *reinterpret_cast<volatile int *>(err) == ERR_TIMEOUT)) {
                         if (lane == 0) atomicCAS(err, 0, ERR_TIMEOUT);
                         drain = true;
                     }
@@ -1051,7 +1052,7 @@ cudaError_t launch_round(const EdgeDesc *edges, const NodeDesc *nodes, int n_nod
                          const InRec *in_rec, const int *order, const int *model_node_off, const int *model_edge_off,
                          int n_models, const float *tab, const ulonglong2 *agg, const ulonglong2 *msg, const float *un0,
                          int *labels, double *energy, int *err, int max_label, int max_terms, double *part,
-                         cudaStream_t st)
+                         long long spin_limit, int test_wait, cudaStream_t st)
 {
     if (max_label <= 32 * 4 * kRoundMaxWarps) {
         // labels and the queue's counter behind them: -1
@@ -1069,7 +1070,7 @@ cudaError_t launch_round(const EdgeDesc *edges, const NodeDesc *nodes, int n_nod
         const int per_sm = 1536 / threads;            // enough to fill an SM; any grid is safe
         const int blocks = static_cast<int>(std::min<long long>((n_nodes + teams - 1) / teams, 152LL * per_sm));
         kernel<<<blocks, threads, 0, st>>>(nodes, order, n_nodes, in_off, in_rec, tab, agg, msg, labels,
-                                           labels + n_nodes, err);
+                                           labels + n_nodes, err, spin_limit, test_wait);
     } else {
         round_kernel<<<n_models, kRoundThreads, 0, st>>>(nodes, in_off, in_rec, model_node_off, tab, agg, msg, labels,
                                                          err);

@@ -206,12 +206,13 @@ cudaError_t launch_bound(const EdgeDesc *edges, int n_edges, const NodeDesc *nod
 // Primal rounding, then the energies.  order: the nodes by level of the
 // rounding order (a node's earlier neighbours lie in lower levels); labels has
 // room for one entry more (the queue's counter); max_label: the largest label
-// count.
+// count; spin_limit: polls of a wait for a label; test_wait: testing (the last
+// node waits for labels that it never sees).
 cudaError_t launch_round(const EdgeDesc *edges, const NodeDesc *nodes, int n_nodes, const int *in_off,
                          const InRec *in_rec, const int *order, const int *model_node_off, const int *model_edge_off,
                          int n_models, const float *tab, const ulonglong2 *agg, const ulonglong2 *msg, const float *un0,
                          int *labels, double *energy, int *err, int max_label, int max_terms, double *part,
-                         cudaStream_t st);
+                         long long spin_limit, int test_wait, cudaStream_t st);
 int sum_slices(int max_terms);  // partial sums per model of a sum over its edges and nodes (> 1: one launch more)
 // stamp[0]: nonzero if a state entry may carry a version other than 0.  A full
 // pack (stamp given) and a reset clear it; who lets a kernel write versions

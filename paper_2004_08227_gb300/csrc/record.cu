@@ -563,7 +563,8 @@ __global__ void __launch_bounds__(4 * grp_labels<NC>(), grp_blocks<NC>())
             if (vt < Lv) vh[vt] = x = bw_poll_diff(p, p.agg + ed.av + vt, p.msg + ed.mv + vt, vv, ve, drain);
             shifted(0, vt, Lv, x, 0.f);
         }
-        if (warp >= W - V && ut < Lu) uh[ut] = bw_poll_diff(p, p.agg + ed.au + ut, p.msg + ed.mu + ut, vu, ve, drain);
+        if (warp >= W - V && ut < Lu)
+            uh[ut] = bw_poll_diff(p, p.agg + ed.au + ut, p.msg + ed.mu + ut, g > 0 ? vu : vu + p.test_wait, ve, drain);
         __syncthreads();
         const long long g2 = s_g[(turn + 1) & 1];
         int4 nrec = make_int4(0, 0, 0, 0);

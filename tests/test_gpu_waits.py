@@ -13,8 +13,10 @@ TIMEOUT = -4
 
 
 def _tied(n, labels, seed):
-    """K_n with integer costs (exact ties); its first edge leads to its last node."""
-    m = W.uneven_complete(n, max(1, labels - 3), labels, seed=seed)
+    """K_n with integer costs (exact ties); its first edge leads to its last node,
+    which alone has more than 300 labels."""
+    m = W.uneven_complete(n, max(1, min(labels, 300) - 3), min(labels, 300), seed=seed)
+    m.labels[-1] = labels
     k = np.random.default_rng(seed).permutation(m.E)
     k = np.concatenate([[m.E - 1], k[k != m.E - 1]])
     size = int((m.labels[m.edge_u].astype(np.int64) * m.labels[m.edge_v]).sum())
@@ -50,3 +52,49 @@ def test_a_low_limit_leaves_the_automatic_structured_driver_alone():
         b.run(20)
         a.sync()
         assert all(np.array_equal(x, y) for x, y in zip(a.state_arrays()[1:], b.state_arrays()[1:]))
+
+
+def _raises_timeout(call):
+    with pytest.raises(MplppError) as ei:
+        call()
+    assert ei.value.status == TIMEOUT
+
+
+@pytest.mark.parametrize("n,labels", [(2, 5), (30, 16), (20, 40), (12, 70), (4, 1025)])
+def test_a_wait_of_the_rounding_runs_out(n, labels):
+    """One team waits for a label that it never sees; the next call on the same
+    solver, and another solver, work."""
+    m = _tied(n, labels, n)
+    with Solver([m], mode="looped", test_unreachable_wait=True, spin_limit=2000) as s, Solver([m], mode="looped") as good:
+        s.run(1)
+        _raises_timeout(s.labeling)
+        good.run(1)
+        assert np.array_equal(s.bound(), good.bound())
+        x, _ = good.labeling()
+        assert (x >= 0).all() and (x < m.labels).all()
+
+
+@pytest.mark.parametrize("n,labels", [(6, 8), (6, 40), (5, 100), (3, 260)])
+@pytest.mark.parametrize("fp64_replay", [False, True])
+def test_a_wait_of_the_backward_runs_out(n, labels, fp64_replay):
+    """The replay's queue (up to 128 labels), or with the all-FP64 replay, which
+    waits for nothing, the sweep's."""
+    m = W.complete(n, labels, seed=1)
+    with Solver([m], mode="looped", record_every=2, test_unreachable_wait=True, spin_limit=2000,
+                test_fp64_replay=fp64_replay) as s:
+        s.run(3)
+        _raises_timeout(s.backward)
+        s.reset()
+        s.run(1)
+        s.sync()
+
+
+@pytest.mark.parametrize("how", ["labeling", "backward"])
+def test_a_low_limit_leaves_the_rounding_and_the_backward_alone(how):
+    m = W.uneven_complete(40, 2, 30, seed=2)
+    with Solver([m], mode="looped", record_every=2, spin_limit=1) as a, \
+            Solver([m], mode="looped", record_every=2) as b:
+        a.run(3)
+        b.run(3)
+        x, y = (a.labeling(), b.labeling()) if how == "labeling" else (a.backward(), b.backward())
+        assert all(np.array_equal(p, q) for p, q in zip(x, y))
