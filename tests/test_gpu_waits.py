@@ -98,3 +98,34 @@ def test_a_low_limit_leaves_the_rounding_and_the_backward_alone(how):
         b.run(3)
         x, y = (a.labeling(), b.labeling()) if how == "labeling" else (a.backward(), b.backward())
         assert all(np.array_equal(p, q) for p, q in zip(x, y))
+
+
+def _star(labels):
+    rng = np.random.default_rng(7)
+    labels = np.asarray(labels, np.int32)
+    n = labels.shape[0]
+    eu, ev = np.zeros(n - 1, np.int32), np.arange(1, n, dtype=np.int32)
+    size = int((labels[eu].astype(np.int64) * labels[ev]).sum())
+    return W.Model(labels, eu, ev, rng.random(int(labels.sum())).astype(np.float32),
+                   rng.standard_normal(size).astype(np.float32))
+
+
+@pytest.mark.parametrize("name,kw", [
+    ("k10", {"cluster": 1, "threads": 128}),  # a CTA per edge, rows in registers
+    ("k10", {"cluster": 2, "threads": 128}),  # a cluster per edge
+    ("k10_40", {}),                           # the automatic mapping above 32 labels
+    ("star_132", {"cluster": 1, "threads": 512}),             # wide rows, with a warp that polls
+    ("k10", {}),                              # the narrow form
+])
+def test_a_wait_of_the_persistent_drivers_runs_out(name, kw):
+    models = {"k10": lambda: W.complete(10, 8, seed=0), "k10_40": lambda: W.complete(10, 40, seed=0),
+              "star_132": lambda: _star([40, 132, 132, 130, 131])}
+    m = models[name]()
+    with Solver([m], mode="persistent", test_unreachable_wait=True, spin_limit=2000, **kw) as s:
+        assert s.info()["poller_warp"] == int(name == "star_132")
+        s.run(3)
+        _raises_timeout(s.sync)
+    with Solver([m], mode="persistent", **kw) as s, Solver([m], mode="looped") as ref:
+        s.run(3)
+        ref.run(3)
+        assert all(np.array_equal(x, y) for x, y in zip(s.state_arrays()[1:], ref.state_arrays()[1:]))
