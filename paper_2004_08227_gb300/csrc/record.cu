@@ -11,7 +11,6 @@
 // One CTA per edge of a matching; one launch per matching (label counts up to
 // 128: one launch for all iterations, rec_queue_kernel).
 #include <algorithm>
-#include <cfloat>
 #include <climits>
 
 #include "backward.h"
@@ -437,7 +436,7 @@ __host__ __device__ inline int grp_stride(int ld)  // words, = 8 mod 32, >= ld
 
 // Argmin of one line from its 4 lanes' screen sums: sv[r] <= thr are the
 // candidates, index(r) their positions, value(j) the FP64 value at position j.
-// Valid in every lane of the line.
+// Valid in every lane of the line; INT_MAX without a candidate.
 template <int N, typename Index, typename Value>
 __device__ __forceinline__ int line_argmin(const float (&sv)[N], float thr, Index index, Value value)
 {
@@ -445,7 +444,7 @@ __device__ __forceinline__ int line_argmin(const float (&sv)[N], float thr, Inde
     unsigned m = 0u;
 #pragma unroll
     for (int r = 0; r < N; ++r)
-        if (sv[r] <= thr) m |= 1u << r;  // +inf beyond the line; thr is less
+        if (sv[r] <= thr) m |= 1u << r;  // +inf beyond the line; thr is finite
     int cnt = __popc(m);
     cnt += __shfl_xor_sync(kAll, cnt, 1);
     cnt += __shfl_xor_sync(kAll, cnt, 2);
@@ -479,13 +478,31 @@ __device__ __forceinline__ int line_argmin(const float (&sv)[N], float thr, Inde
     return arg;
 }
 
-// The screen's threshold from the line's smallest sum, rounded upwards, finite.
+// The screen's threshold from the line's smallest sum, rounded upwards.  From
+// 2^125 on a sum may overflow that the FP64 minimum does not exceed (or all of
+// them, as in a table of 1.7e38 against a vector of 1.8e38): no candidate then.
 __device__ __forceinline__ float line_threshold(float mn, float d)
 {
     mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, 1));
     mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, 2));
     const float e4 = __fadd_ru(__fmul_ru(0x1p-20f, __fadd_ru(fabsf(mn), d)), 0x1p-122f);
-    return fminf(__fadd_ru(mn, e4), FLT_MAX);
+    return e4 < 0x1p105f ? __fadd_ru(mn, e4) : -INFINITY;
+}
+
+// Argmin of a line without a candidate: all of it in FP64, by one thread.
+__device__ __forceinline__ int line_argmin_all(const float *th, int stride, const double *x, int n)
+{
+    unsigned long long key = ~0ull;
+    int arg = 0;
+#pragma unroll 1
+    for (int j = 0; j < n; ++j) {
+        const unsigned long long v = order_key(d_of_f(th[j * stride]) + x[j]);
+        if (v < key) {
+            key = v;
+            arg = j;
+        }
+    }
+    return arg;
 }
 
 template <int NC>
@@ -593,8 +610,9 @@ __global__ void __launch_bounds__(4 * grp_labels<NC>(), grp_blocks<NC>())
                 sv, i < Lu ? thr : -INFINITY, [&](int r) { return 4 * (k + 4 * (r >> 2)) + (r & 3); },
                 [&](int j) { return d_of_f(st_i[j]) + x[j]; });
             if (k == 0 && i < Lu) {
-                arg[i] = a == INT_MAX ? 0 : a;
-                if (REC) out[i] = static_cast<unsigned short>(a == INT_MAX ? 0 : a);
+                const int j = a == INT_MAX ? line_argmin_all(st_i, 1, x, Lv) : a;
+                arg[i] = j;
+                if (REC) out[i] = static_cast<unsigned short>(j);
             }
         };
         // pass 1: a(s) = 1/2 (min_t [theta(s,t) + vh(t)] + uh(s)),  alpha = uh - a
@@ -625,8 +643,9 @@ __global__ void __launch_bounds__(4 * grp_labels<NC>(), grp_blocks<NC>())
                 sv, i < Lv ? thr : -INFINITY, [&](int r) { return k + 4 * r; },
                 [&](int j) { return d_of_f(st[j * ldp + i]) + al[j]; });
             if (k == 0 && i < Lv) {
-                arg[i] = a == INT_MAX ? 0 : a;
-                if (REC) s2[i] = static_cast<unsigned short>(a == INT_MAX ? 0 : a);
+                const int j = a == INT_MAX ? line_argmin_all(st + i, ldp, al, Lu) : a;
+                arg[i] = j;
+                if (REC) s2[i] = static_cast<unsigned short>(j);
             }
         }
         __syncthreads();
