@@ -3,7 +3,6 @@
 // A warp walks a fixed list of steps in schedule order, each up to 32 / LM edges
 // of one matching; an edge belongs to the same lanes in every iteration.
 //
-//
 // One warp per block.  As in the persistent driver of handshake.cu the state
 // lives in versioned entries (common.cuh): a lane polls the two node entries of
 // its label until they carry the update count it expects, and the new entries
@@ -15,13 +14,15 @@
 // Bound by the chain from one matching to the next: a store and a polling round
 // trip through L2, then the update.  What else a step needs -- its table, the
 // edge's messages, which the same lanes wrote an iteration ago, and its record --
-// is copied into shared memory two steps ahead by cp.async.  K_600 with 13
-// labels, per matching: 2.44 us with a CTA of 128 threads per edge, 1.53 us with
-// these loads prefetched into registers (a warp has six load scoreboards: its
-// wait for the node entries took in the prefetches behind them), 1.15 us so.
-// Node vectors in the distributed shared memory of a cluster of 16 CTAs, with a
-// cluster barrier per matching, took 1.86 us: 16 SMs issue too slowly for 300
-// edges.
+// is copied into shared memory two steps ahead by cp.async (the messages only
+// where the copy comes a step or more after they were stored, which a warp
+// barrier separates: with one or two steps in an iteration they are loaded at
+// their turn).  K_600 with 13 labels, per matching: 2.44 us with a CTA of 128
+// threads per edge, 1.53 us with these loads prefetched into registers (a warp
+// has six load scoreboards: its wait for the node entries took in the prefetches
+// behind them), 1.15 us so. Node vectors in the distributed shared memory of a
+// cluster of 16 CTAs, with a cluster barrier per matching, took 1.86 us: 16 SMs
+// issue too slowly for 300 edges.
 #include <cfloat>
 #include <cstdint>
 
@@ -87,7 +88,7 @@ struct Walk {
 #pragma unroll
         for (int j = 0; j < LM / 4; ++j)
             if (l + j * LM < chunks) cp_async16(dst + 4 * (l + j * LM), src + 4 * (l + j * LM));
-        if (n > 1) {  // phi_{v->u}, then phi_{u->v}: one run of entries
+        if (n > 2) {  // phi_{v->u}, then phi_{u->v}: one run of entries
             const int entries = ((Lu + 3) & ~3) + ((Lv + 3) & ~3);
 #pragma unroll
             for (int j = 0; j < 2; ++j)
@@ -127,10 +128,10 @@ struct Walk {
             for (int s = 0; s < LM; ++s) col[s] = s < r.Lu ? th[s * r.ld + t0] : INFINITY;
         }
         ulonglong2 xu = make_ulonglong2(0ull, 0ull), xv = xu;
-        if (n > 1) {
+        if (n > 2) {
             if (l < r.Lu) xu = st.msg[k & 1][l];
             if (l < r.Lv) xv = st.msg[k & 1][((r.Lu + 3) & ~3) + l];
-        } else {  // the step before is the same edge's: its new messages
+        } else {  // this edge's step came one or two before: its new messages, by the lanes that stored them
             if (l < r.Lu) xu = ld_se(msg + r.mu + l);
             if (l < r.Lv) xv = ld_se(msg + r.mv + l);
         }
