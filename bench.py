@@ -107,6 +107,25 @@ def kernel_traffic(iterations):
         return None
 
 
+def run_launches(info, iterations):
+    """Kernel launches of one run (info: Solver.info()): one per matching and
+    iteration, or one kernel for all of them, before which every driver but the
+    resident one clears the state's versions."""
+    if info["launches_per_iteration"]:
+        return iterations * info["launches_per_iteration"]
+    return 1 if info["mode"] == "resident" else 2
+
+
+def run_kernel(info):
+    """The kernel that a run launches."""
+    if info["mode"] == "persistent":  # cluster 0: the form for small label counts
+        return "hs_persistent_kernel" if info["cluster"] else "hs_narrow_kernel"
+    if info["mode"] == "structured":
+        return "struct_kernel" if info["launches_per_iteration"] else "struct_queue_kernel"
+    return {"queue": "hs_queue_kernel", "resident": "hs_resident_kernel", "warp": "hs_warp_kernel",
+            "structured_queue": "struct_queue_kernel"}.get(info["mode"], "hs_looped_kernel")
+
+
 def load_peak():
     p = os.path.join(ROOT, "MEASURED_PEAKS.json")
     try:
@@ -647,9 +666,7 @@ def run_ours(args):
     achieved = T * bytes_iter / (kms / 1e3) / 1e9
     achieved32 = T * bytes_iter32 / (kms / 1e3) / 1e9
     peak, peak_kind = load_peak()
-    kernel = {"persistent": "hs_persistent_kernel", "queue": "hs_queue_kernel", "resident": "hs_resident_kernel",
-              "warp": "hs_warp_kernel", "structured": "struct_kernel",
-              "structured_queue": "struct_queue_kernel"}.get(info["mode"], "hs_looped_kernel")
+    kernel = run_kernel(info)
 
     # the looped driver (one launch per matching) on the same workload, equal bound
     looped = None
@@ -718,12 +735,10 @@ def run_ours(args):
                "h2d_bytes_per_step": int(h2d), "d2h_bytes_per_step": int(d2h), "ms_per_step": et * 1e3,
                "step_ms": [round(t * 1e3, 2) for t in times], "timer": "host wall clock"}
 
-    # per step: reset (1), the run (restamp + one persistent launch, or one
-    # launch per matching and iteration), exact bound (the scan and the sum, one
-    # more where the sum runs in slices), rounding + energy
+    # per step: reset (1), the run, exact bound (the scan and the sum, one more
+    # where the sum runs in slices), rounding + energy
     bound_launches = 2 + int(max(m.n + m.E for m in models) >= 4096)
-    launches_per_step = (1 + (2 if info["mode"] in ("persistent", "warp", "queue") else T * info["phases"])
-                         + bound_launches + info["labeling_launches"])
+    launches_per_step = 1 + run_launches(info, T) + bound_launches + info["labeling_launches"]
     line = {
         "metric": "edge_updates_per_s", "value": value, "unit": "edge_updates/s", "n_gpus": world,
         "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms, "higher_is_better": True,
@@ -736,7 +751,7 @@ def run_ours(args):
         "hbm_gbs": achieved,
         "roofline": {"bound": "hbm", "kernel": kernel, "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "peak_source": peak_kind,
-                     "traffic": kernel_traffic(T) if (cfg == 2 and info["mode"] == "persistent") else None,
+                     "traffic": kernel_traffic(T) if (cfg == 2 and kernel == "hs_persistent_kernel") else None,
                      "algorithmic_bytes_per_launch": T * bytes_iter,
                      "bytes_formula": "per edge update 4 L_u L_v + 16 (L_u + L_v)",
                      "achieved_state32": achieved32, "frac_state32": achieved32 / peak,
