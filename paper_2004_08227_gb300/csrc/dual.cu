@@ -135,8 +135,7 @@ __global__ void __launch_bounds__(kThreads) pack_kernel(PackPtrs ptrs, int model
 // collected over a warp's edges and evaluated 32 at a time: an FP64 instruction
 // holds the pipe for a whole warp however few lanes are active.  For the same
 // reason floats are widened by integer operations: four FP64 instructions per
-// 32 entries instead of nine (kNN, 57,000 tables of 64 x 64: 256 -> 231 us;
-// 2,048 K_20, 8 labels: 315 -> 295 us; K_600, 13 labels: 228 -> 198 us).  They
+// 32 entries instead of nine (kNN, 57,000 tables of 64 x 64: 256 -> 231 us).  They
 // meet in emin by atomicMin, so emin must hold ~0 before (bound_sum_kernel leaves
 // it so).
 struct Final {  // an entry to evaluate in FP64
@@ -531,7 +530,7 @@ __global__ void __launch_bounds__(TEAM ? 32 * kRoundMaxWarps : 32 * kRoundWarps)
                 unsigned ready = __ballot_sync(kAll, x >= 0) & pending;
                 if (!ready) {
                     if (!TEAM && !fetched && __popc(pending) <= kRoundFetch) {
-                        // their tables (at most 64 KB each) and messages into L2
+                        // their tables (at most 16 KB each) and messages into L2
                         fetched = true;
                         for (unsigned left = pending; left; left &= left - 1u) {
                             const int src = __ffs(left) - 1;
